@@ -94,7 +94,7 @@ def main(argv=None):
     ap.add_argument("--precision", default="fp64", choices=["fp64", "bf16x3", "tf32x3"])
     ap.add_argument("--scale", type=float, default=None, help="override the factor entry scale")
     ap.add_argument("--no-diis-t3", action="store_true", help="DIIS on T1 and T2 only")
-    ap.add_argument("--f64-tc", type=int, default=0, choices=[0, 1, 2],
+    ap.add_argument("--f64-tc", type=int, default=0, choices=[0, 1, 2, 3],
                     help="FP64 contractions on the tensor cores (option f64_tc)")
     ap.add_argument("--solve", action="store_true", help="iterate to --tol with rccsdt_solve")
     ap.add_argument("--tol", type=float, default=1e-8)
