@@ -336,9 +336,11 @@ template void launch_r3_gather<double>(const float*, const i64*, int, const int*
 //
 // The FP64 pipe takes about 2 FMA per clock and SM and bounds everything here: a 16 x 16
 // tile costs 128 clocks per k against about 4 for gathering its 32 operand values, so
-// tiles are small -- little padding on ragged edges, and enough of them to reach every
-// SM -- and the gathers, repeated per tile, stay hidden.  (64 x 64 tiles left one CTA
-// 2048 clocks per k: at o = 3, v = 12 a contraction took 48 us, and its two panel
+// tiles are small: little padding on ragged edges, and enough of them to reach every
+// SM.  From panels they run at the pipe's rate (1176 x 2688 x 1176: 6.07 ms; 64 x 64 tiles
+// 7.1).  Gathers are repeated per tile and leave 50 to 80 % of it, so only small contractions
+// gather here (kF64PackFma): for those the launches count.  (64 x 64 tiles of panels left one
+// CTA 2048 clocks per k: at o = 3, v = 12 a contraction took 48 us, and its two panel
 // gathers 7 us each.)  Outputs with at most four rows or columns use 4 x 64 tiles.  With
 // few tiles K is split over the CTAs of a cluster, whose partial tiles are added through
 // distributed shared memory in rank order, or, beyond 8 slices, over global partials.
