@@ -151,26 +151,23 @@ int gproblem_tiles(const GProblem& p);
 // Cuts K into slices of `len` K values (a multiple of 64); the number of slices.
 int split_gproblem(GProblem* p, int len);
 int gemm_tc_block_k(int kind, int bn);
-// One persistent launch over every tile of the nprob problems (device table,
-// tile0 prefix order, tables made with the same bn); grid <= 0 picks one CTA per SM.
 // FP64-accurate GEMM on the BF16 tensor cores (digit planes, see elem.cuh):
 // launch_slice_f64 cuts an FP64 panel [R][Kpad] into kSlices BF16 planes
-// [kSlices][R][Kpad] and one scale exponent per row; launch_gemm_f64e then applies
-// the table epilogue e (FP64 or FP32 outputs, FP64 arithmetic) to the product of two such panels.
+// [kSlices][R][Kpad] and one scale exponent per row, launch_slice_f64x into kSlicesX;
+// launch_gemm_f64e then applies the table epilogue e (FP64 or FP32 outputs, FP64 arithmetic) to
+// the product of two such panels of ns planes.  K is split over the SMs when there are few
+// tiles (partial sums in `scratch`, scratch_elems doubles, null: no split).  With `raw` the
+// product itself is stored, column-major [N][M], and e only gives M and N.
 // Kpad a multiple of 64.  Returns nonzero for an unsupported configuration.
 void launch_slice_f64(const double* P, int R, int Kpad, void* planes, int* exps, cudaStream_t s);
-int launch_gemm_f64e(const void* Aplanes, const int* ea, const void* Bplanes, const int* eb, int Kpad, const EpiArgs& e,
-                     int* status_flag, long long watchdog, cudaStream_t s);
-// The same with kSlicesX planes (full FP64 operand width), and the product of panels of
-// ns planes with K split over the SMs when there are few tiles (partial sums in
-// `scratch`, scratch_elems doubles, null: no split).  With `raw` the product itself is
-// stored, column-major [N][M], and e only gives M and N.
 void launch_slice_f64x(const double* P, int R, int Kpad, void* planes, int* exps, cudaStream_t s);
-int launch_gemm_f64e_split(const void* Aplanes, const int* ea, const void* Bplanes, const int* eb, int Kpad, int ns,
-                           const EpiArgs& e, int* status_flag, long long watchdog, double* scratch, i64 scratch_elems,
-                           cudaStream_t s, double* raw = nullptr);
+int launch_gemm_f64e(const void* Aplanes, const int* ea, const void* Bplanes, const int* eb, int Kpad, int ns,
+                     const EpiArgs& e, int* status_flag, long long watchdog, double* scratch, i64 scratch_elems,
+                     cudaStream_t s, double* raw = nullptr);
 // C (epilogue e) += the sum over z, in order, of partial[z][M][N].
 void launch_splitk_reduce(const double* partial, int splitk, const EpiArgs& e, cudaStream_t s);
+// One persistent launch over every tile of the nprob problems (device table,
+// tile0 prefix order, tables made with the same bn); grid <= 0 picks one CTA per SM.
 int launch_gemm_tc_grouped(int kind, const GProblem* probs, int nprob, int total_tiles, int grid, int bn,
                            int* status_flag, long long watchdog, cudaStream_t s);
 // The same with the tile count and every problem's tile0 read from device memory

@@ -17,6 +17,8 @@
 namespace rcc {
 
 long long g_launch_count = 0;
+// launches by form (test hook): gathering products, grouped FP64 products, grouped split products, grouped combines
+long long g_forms[4] = {0, 0, 0, 0};
 
 void launch_pack(const PackArgs& a, cudaStream_t) {
   for (int r = 0; r < a.R; ++r)
@@ -37,6 +39,35 @@ void launch_gemm_f64(const double* A, const double* B, int K, int lda, int ldb, 
       for (int k = 0; k < K; ++k) s += A[(i64)m * lda + k] * B[(i64)n * ldb + k];
       epi_apply(e, m, n, s);
     }
+}
+
+static double host_operand(const PackArgs& a, const double* panel, int r, int k) {
+  return panel ? panel[(i64)r * a.Kpad + k] : pack_value(a, r, k);
+}
+void launch_gemm_f64_gather(const PackArgs& a, const double* Apanel, const PackArgs& b, const double* Bpanel, int K,
+                            const EpiArgs& e, double*, i64, cudaStream_t) {
+  ++g_forms[0];
+  for (int m = 0; m < e.M; ++m)
+    for (int n = 0; n < e.N; ++n) {
+      double s = 0.0;
+      for (int k = 0; k < K; ++k) s += host_operand(a, Apanel, m, k) * host_operand(b, Bpanel, n, k);
+      epi_apply(e, m, n, s);
+    }
+}
+
+int f64_product_tiles(const F64Product& p) { return (p.M + 15) / 16 * ((p.N + 15) / 16) * p.slices; }
+void launch_gemm_f64_grouped(const F64Product* list, int n, int, cudaStream_t) {
+  ++g_forms[1];
+  for (int q = 0; q < n; ++q) {
+    const F64Product& p = list[q];
+    for (int z = 0; z < p.slices; ++z)
+      for (int m = 0; m < p.M; ++m)
+        for (int nn = 0; nn < p.N; ++nn) {
+          double s = 0.0;
+          for (int k = z * p.kz; k < std::min(p.K, (z + 1) * p.kz); ++k) s += pack_value(p.a, m, k) * pack_value(p.b, nn, k);
+          p.out[((i64)z * p.M + m) * p.N + nn] = s;
+        }
+  }
 }
 
 // Split-precision product hi*hi + hi*lo + lo*hi with float products and a float
@@ -77,6 +108,32 @@ void launch_combine(const CombineArgs& c, cudaStream_t) {
     double s = c.beta == 0.0 ? 0.0 : c.beta * c.out[ooff];
     for (int t = 0; t < c.nterm; ++t) s += c.coef[t] * c.in[t][ioff[t]];
     c.out[ooff] = s;
+  }
+}
+
+void prepare_apply(ApplyArgs*) {}
+void launch_apply_grouped(const ApplyArgs* list, const int*, int n, int, int, cudaStream_t s) {
+  ++g_forms[3];
+  for (int q = 0; q < n; ++q) {
+    const ApplyArgs& a = list[q];
+    launch_combine(a.c, s);
+    for (i64 idx = 0; idx < a.c.total; ++idx) {
+      i64 rem = idx, ooff = 0, roff[kMaxRaw] = {};
+      for (int d = a.c.rank - 1; d >= 0; --d) {
+        const i64 x = rem % a.c.shape[d];
+        rem /= a.c.shape[d];
+        ooff += x * a.c.ostride[d];
+        for (int t = 0; t < a.nraw; ++t) roff[t] += x * a.rstride[t][d];
+      }
+      for (int t = 0; t < a.nraw; ++t) {
+        double y = 0.0;
+        for (int z = 0; z < a.splitk[t]; ++z) {
+          const i64 at = roff[t] + z * a.slice[t];
+          y += a.wide ? ((const double*)a.raw[t])[at] : (double)a.raw[t][at];
+        }
+        a.c.out[ooff] += a.alpha[t] * y;
+      }
+    }
   }
 }
 
@@ -235,7 +292,8 @@ void launch_r1_cubes_reduce(const float* part, int ppz, int nz, int v, double* d
     }
 }
 
-void launch_slice_f64(const double* P, int R, int Kpad, void* planes, int* exps, cudaStream_t) {
+template <int NS>
+static void host_slice(const double* P, int R, int Kpad, void* planes, int* exps) {
   __nv_bfloat16* pl = (__nv_bfloat16*)planes;
   const i64 plane = (i64)R * Kpad;
   for (int r = 0; r < R; ++r) {
@@ -243,30 +301,39 @@ void launch_slice_f64(const double* P, int R, int Kpad, void* planes, int* exps,
     for (int k = 0; k < Kpad; ++k) mx = std::max(mx, f64_magnitude_bits(P[(i64)r * Kpad + k]));
     exps[r] = slice_exponent(mx);
     for (int k = 0; k < Kpad; ++k) {
-      float a[kSlices];
+      float a[NS];
       slice_digits(P[(i64)r * Kpad + k], exps[r], a);
-      for (int s = 0; s < kSlices; ++s) pl[s * plane + (i64)r * Kpad + k] = __float2bfloat16_rn(a[s]);
+      for (int s = 0; s < NS; ++s) pl[s * plane + (i64)r * Kpad + k] = __float2bfloat16_rn(a[s]);
     }
   }
 }
+void launch_slice_f64(const double* P, int R, int Kpad, void* planes, int* exps, cudaStream_t) {
+  host_slice<kSlices>(P, R, Kpad, planes, exps);
+}
+void launch_slice_f64x(const double* P, int R, int Kpad, void* planes, int* exps, cudaStream_t) {
+  host_slice<kSlicesX>(P, R, Kpad, planes, exps);
+}
 
-// The digit products with s + t <= 5, summed in FP64 (the device sums them exactly,
-// up to the FP32 rounding of the smallest ones).
-int launch_gemm_f64e(const void* Aplanes, const int* ea, const void* Bplanes, const int* eb, int Kpad, const EpiArgs& e,
-                     int*, long long, cudaStream_t) {
+// The digit products with s + t <= 5 (six planes) or 7 (seven), summed in FP64 (the device
+// sums them exactly, up to the FP32 rounding of the smallest ones).
+int launch_gemm_f64e(const void* Aplanes, const int* ea, const void* Bplanes, const int* eb, int Kpad, int ns,
+                     const EpiArgs& e, int*, long long, double*, i64, cudaStream_t, double* raw) {
   if (Kpad % 64 != 0) return 1;
   const __nv_bfloat16* A = (const __nv_bfloat16*)Aplanes;
   const __nv_bfloat16* B = (const __nv_bfloat16*)Bplanes;
   const i64 pa = (i64)e.M * Kpad, pb = (i64)e.N * Kpad;
+  const int last = ns == kSlicesX ? 7 : 5;
   for (int m = 0; m < e.M; ++m)
     for (int n = 0; n < e.N; ++n) {
       double s = 0.0;
       for (int k = 0; k < Kpad; ++k)
-        for (int sa = 0; sa < kSlices; ++sa)
-          for (int sb = 0; sb + sa < kSlices; ++sb)
+        for (int sa = 0; sa < ns; ++sa)
+          for (int sb = 0; sb < ns && sb + sa <= last; ++sb)
             s += (double)__bfloat162float(A[sa * pa + (i64)m * Kpad + k]) *
                  (double)__bfloat162float(B[sb * pb + (i64)n * Kpad + k]);
-      epi_apply(e, m, n, std::ldexp(s, ea[m] + eb[n] - 14));
+      s = std::ldexp(s, ea[m] + eb[n] - 14);
+      if (raw) raw[(i64)n * e.M + m] = s;
+      else epi_apply(e, m, n, s);
     }
   return 0;
 }
@@ -276,12 +343,12 @@ void launch_zero_cols(const CubeDst& d, i64 rows, int k0, int kind, cudaStream_t
     for (int k = k0; k < d.Kpad; ++k) host_store_split(kind, d.out_hi, d.out_lo, r * d.Kpad + k, 0.f);
 }
 
-int gemm_tc_block_k(int kind) { return kind == PANEL_BF16X2 ? 64 : 32; }
+int gemm_tc_block_k(int kind, int) { return kind == PANEL_BF16X2 ? 64 : 32; }
 
 int make_gproblem(GProblem* p, int kind, const void* Ahi, const void* Alo, const void* Bhi, const void* Blo, int M,
                   int N, int Kpad, float* out, int bn) {
   if (kind != PANEL_BF16X2 && kind != PANEL_TF32X2) return 1;
-  if (Kpad % gemm_tc_block_k(kind) != 0 || M <= 0 || N <= 0) return 1;
+  if (Kpad % gemm_tc_block_k(kind, 256) != 0 || M <= 0 || N <= 0) return 1;
   memset((void*)p, 0, sizeof(*p));
   p->colmajor = 0;
   p->a_hi = Ahi;
@@ -292,24 +359,42 @@ int make_gproblem(GProblem* p, int kind, const void* Ahi, const void* Alo, const
   p->M = M;
   p->N = N;
   p->Kpad = Kpad;
-  p->kblocks = Kpad / gemm_tc_block_k(kind);
+  p->kblocks = Kpad / gemm_tc_block_k(kind, 256);
   p->mt = (M + 127) / 128;
   p->nt = (N + (bn == 128 ? 127 : 255)) / (bn == 128 ? 128 : 256);
+  p->splitk = 1;
+  p->kb_per = p->kblocks;
   return 0;
 }
 
-int gproblem_tiles(const GProblem& p) { return p.mt * p.nt; }
+int gproblem_tiles(const GProblem& p) { return p.mt * p.nt * p.splitk; }
 
-int launch_gemm_tc_grouped(int kind, const GProblem* probs, int nprob, int, int, int, int* flag, long long wd,
-                           cudaStream_t s) {
+int split_gproblem(GProblem* p, int len) {
+  const int bk = p->Kpad / p->kblocks;
+  p->kb_per = std::max(1, std::min(p->kblocks, len / bk));
+  p->splitk = (p->kblocks + p->kb_per - 1) / p->kb_per;
+  return p->splitk;
+}
+
+int launch_gemm_tc_grouped(int kind, const GProblem* probs, int nprob, int, int, int, int*, long long, cudaStream_t) {
+  ++g_forms[2];
+  auto get = [&](const void* p, i64 i) -> float {
+    return kind == PANEL_BF16X2 ? __bfloat162float(((const __nv_bfloat16*)p)[i]) : ((const float*)p)[i];
+  };
   for (int q = 0; q < nprob; ++q) {
     const GProblem& P = probs[q];
-    EpiArgs e{};
-    e.M = P.M;
-    e.N = P.N;
-    if (launch_gemm_tc(kind, P.a_hi, P.a_lo, P.b_hi, P.b_lo, P.Kpad, e, flag, wd, s, nullptr, 0, P.out, 256,
-                       P.colmajor))
-      return 1;
+    const int len = P.Kpad / P.kblocks * P.kb_per;
+    for (int z = 0; z < P.splitk; ++z)
+      for (int m = 0; m < P.M; ++m)
+        for (int n = 0; n < P.N; ++n) {
+          float s = 0.f;
+          for (int k = z * len; k < std::min(P.Kpad, (z + 1) * len); ++k) {
+            const i64 ia = (i64)m * P.Kpad + k, ib = (i64)n * P.Kpad + k;
+            const float ah = get(P.a_hi, ia), al = get(P.a_lo, ia), bh = get(P.b_hi, ib), bl = get(P.b_lo, ib);
+            s += ah * bh + ah * bl + al * bh;
+          }
+          P.out[P.colmajor ? (i64)n * P.M + m : ((i64)z * P.M + m) * P.N + n] = s;
+        }
   }
   return 0;
 }
@@ -594,9 +679,9 @@ void launch_r1_t3(const T* S, const double* oovv, int o, int v, double* dR1_z, d
 }
 template void launch_r1_t3<double>(const double*, const double*, int, int, double*, double*, i64, cudaStream_t);
 template void launch_r1_t3<float>(const float*, const double*, int, int, double*, double*, i64, cudaStream_t);
-template <typename T>
-void launch_scatter_rows3(const float* X, int M, int v, const i64* row_base, const int* row_sel,
-                          const double* row_alpha, T* C, cudaStream_t) {
+template <typename TX, typename T>
+static void host_scatter_rows3(const TX* X, int M, int v, const i64* row_base, const int* row_sel,
+                               const double* row_alpha, T* C) {
   const int P[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
   const i64 V3 = (i64)v * v * v, S[3] = {(i64)v * v, v, 1};
   for (int m = 0; m < M; ++m) {
@@ -607,6 +692,20 @@ void launch_scatter_rows3(const float* X, int M, int v, const i64* row_base, con
     }
   }
 }
+template <typename T>
+void launch_scatter_rows3(const float* X, int M, int v, const i64* row_base, const int* row_sel,
+                          const double* row_alpha, T* C, cudaStream_t) {
+  host_scatter_rows3(X, M, v, row_base, row_sel, row_alpha, C);
+}
+template <typename T>
+void launch_scatter_rows3_f64(const double* X, int M, int v, const i64* row_base, const int* row_sel,
+                              const double* row_alpha, T* C, cudaStream_t) {
+  host_scatter_rows3(X, M, v, row_base, row_sel, row_alpha, C);
+}
+template void launch_scatter_rows3_f64<float>(const double*, int, int, const i64*, const int*, const double*, float*,
+                                              cudaStream_t);
+template void launch_scatter_rows3_f64<double>(const double*, int, int, const i64*, const int*, const double*, double*,
+                                               cudaStream_t);
 template void launch_scatter_rows3<float>(const float*, int, int, const i64*, const int*, const double*, float*,
                                           cudaStream_t);
 template void launch_scatter_rows3<double>(const float*, int, int, const i64*, const int*, const double*, double*,
@@ -637,4 +736,11 @@ template void launch_t2_outer<float>(float*, const float*, const float*, const i
 // Test hook: the integer-path binary64 -> binary32 conversion of the panel gathers.
 extern "C" void rcc_test_f64_to_f32(const double* x, float* y, long long n) {
   for (long long i = 0; i < n; ++i) y[i] = rcc::f64_to_f32_rn(x[i]);
+}
+// Test hook: launches by form since the last call.
+extern "C" void rcc_test_forms(long long* out) {
+  for (int q = 0; q < 4; ++q) {
+    out[q] = rcc::g_forms[q];
+    rcc::g_forms[q] = 0;
+  }
 }
