@@ -151,6 +151,35 @@ int gproblem_tiles(const GProblem& p);
 // Cuts K into slices of `len` K values (a multiple of 64); the number of slices.
 int split_gproblem(GProblem* p, int len);
 int gemm_tc_block_k(int kind, int bn);
+// Tile width (in: the wanted one) and K blocks per slice of a split-precision product of its
+// own launch, for launch_gemm_tc and for whoever has to cut K as it does: the FP32 sum of a
+// slice truncates, so its length is part of the result.
+// table: a plain table epilogue, which is bound by its chains of dependent loads (eight warps
+// per tile): with at most half the SMs busy, 128-wide tiles give twice the CTAs and half the
+// epilogue work each.  scratch_elems (0: whole products) bounds the slices' partial tiles.  The
+// split has the shortest critical path: whole waves of tile slices times the K blocks of one
+// slice (plus a few K blocks' worth of epilogue per slice), so that the last wave is not a
+// sliver of the SMs.
+inline int gemm_tc_split(int kind, int M, int N, int Kpad, bool table, long long scratch_elems, int sms, int* bn) {
+  const int mt = (M + 127) / 128;
+  if (*bn != 128 && *bn != 144) *bn = 256;
+  if (*bn == 256 && table && 2LL * mt * ((N + 255) / 256) <= (long long)sms) *bn = 128;
+  const int kblocks = Kpad / gemm_tc_block_k(kind, *bn);
+  const long long tiles = (long long)mt * ((N + *bn - 1) / *bn);
+  if (tiles >= sms || kblocks < 8 || scratch_elems <= 0) return kblocks;
+  long long best = -1;
+  int kb_per = kblocks;
+  for (int sk = 1; sk <= kblocks / 4 && sk <= 64; ++sk) {
+    const int per = (kblocks + sk - 1) / sk, real = (kblocks + per - 1) / per;
+    if (real > 1 && (long long)real * M * N > scratch_elems) break;
+    const long long cost = ((tiles * real + sms - 1) / sms) * (per + 4);
+    if (best < 0 || cost < best) {
+      best = cost;
+      kb_per = per;
+    }
+  }
+  return kb_per;
+}
 // FP64-accurate GEMM on the BF16 tensor cores (digit planes, see elem.cuh):
 // launch_slice_f64 cuts an FP64 panel [R][Kpad] into kSlices BF16 planes
 // [kSlices][R][Kpad] and one scale exponent per row, launch_slice_f64x into kSlicesX;

@@ -70,27 +70,35 @@ void launch_gemm_f64_grouped(const F64Product* list, int n, int, cudaStream_t) {
   }
 }
 
-// Split-precision product hi*hi + hi*lo + lo*hi with float products and a float
-// accumulator (the order of the tensor-core sum is not modelled).
+// Split-precision product hi*hi + hi*lo + lo*hi with float products and a float accumulator
+// per K slice, the slices cut as the device cuts them and added in FP64 (the order of the
+// tensor-core sum is not modelled).
 int launch_gemm_tc(int kind, const void* Ahi, const void* Alo, const void* Bhi, const void* Blo, int Kpad,
-                   const EpiArgs& e, int*, long long, cudaStream_t, float*, long long, float* raw_out, int,
-                   int colmajor) {
+                   const EpiArgs& e, int*, long long, cudaStream_t, float* scratch, long long scratch_elems,
+                   float* raw_out, int bn, int colmajor) {
   auto get = [&](const void* p, i64 i) -> float {
     if (kind == PANEL_BF16X2) return __bfloat162float(((const __nv_bfloat16*)p)[i]);
     return ((const float*)p)[i];
   };
+  const int kb_per = gemm_tc_split(kind, e.M, e.N, Kpad, !raw_out && !e.col_off2,
+                                   scratch && !raw_out ? scratch_elems : 0, 152, &bn);
+  const int len = kb_per * gemm_tc_block_k(kind, bn);
   for (int m = 0; m < e.M; ++m)
     for (int n = 0; n < e.N; ++n) {
-      float s = 0.f;
-      for (int k = 0; k < Kpad; ++k) {
-        const i64 ia = (i64)m * Kpad + k, ib = (i64)n * Kpad + k;
-        const float ah = get(Ahi, ia), al = get(Alo, ia), bh = get(Bhi, ib), bl = get(Blo, ib);
-        s += ah * bh + ah * bl + al * bh;
+      double sum = 0.0;
+      for (int k0 = 0; k0 < Kpad; k0 += len) {
+        float s = 0.f;
+        for (int k = k0; k < std::min(Kpad, k0 + len); ++k) {
+          const i64 ia = (i64)m * Kpad + k, ib = (i64)n * Kpad + k;
+          const float ah = get(Ahi, ia), al = get(Alo, ia), bh = get(Bhi, ib), bl = get(Blo, ib);
+          s += ah * bh + ah * bl + al * bh;
+        }
+        sum += (double)s;
       }
       if (raw_out)
-        raw_out[colmajor ? (i64)n * e.M + m : (i64)m * e.N + n] = s;
+        raw_out[colmajor ? (i64)n * e.M + m : (i64)m * e.N + n] = (float)sum;
       else
-        epi_apply(e, m, n, (double)s);
+        epi_apply(e, m, n, sum);
     }
   return 0;
 }
@@ -343,12 +351,12 @@ void launch_zero_cols(const CubeDst& d, i64 rows, int k0, int kind, cudaStream_t
     for (int k = k0; k < d.Kpad; ++k) host_store_split(kind, d.out_hi, d.out_lo, r * d.Kpad + k, 0.f);
 }
 
-int gemm_tc_block_k(int kind, int) { return kind == PANEL_BF16X2 ? 64 : 32; }
+int gemm_tc_block_k(int kind, int bn) { return (bn == 128 || bn == 144 ? 128 : 64) / (kind == PANEL_BF16X2 ? 2 : 4); }
 
 int make_gproblem(GProblem* p, int kind, const void* Ahi, const void* Alo, const void* Bhi, const void* Blo, int M,
                   int N, int Kpad, float* out, int bn) {
   if (kind != PANEL_BF16X2 && kind != PANEL_TF32X2) return 1;
-  if (Kpad % gemm_tc_block_k(kind, 256) != 0 || M <= 0 || N <= 0) return 1;
+  if (Kpad % gemm_tc_block_k(kind, bn) != 0 || M <= 0 || N <= 0) return 1;
   memset((void*)p, 0, sizeof(*p));
   p->colmajor = 0;
   p->a_hi = Ahi;
@@ -359,7 +367,7 @@ int make_gproblem(GProblem* p, int kind, const void* Ahi, const void* Alo, const
   p->M = M;
   p->N = N;
   p->Kpad = Kpad;
-  p->kblocks = Kpad / gemm_tc_block_k(kind, 256);
+  p->kblocks = Kpad / gemm_tc_block_k(kind, bn);
   p->mt = (M + 127) / 128;
   p->nt = (N + (bn == 128 ? 127 : 255)) / (bn == 128 ? 128 : 256);
   p->splitk = 1;
@@ -743,4 +751,9 @@ extern "C" void rcc_test_forms(long long* out) {
     out[q] = rcc::g_forms[q];
     rcc::g_forms[q] = 0;
   }
+}
+
+// Test hook: the K split of a product's own launch.
+extern "C" int rcc_test_split(int kind, int M, int N, int Kpad, int table, long long scratch, int sms, int* bn) {
+  return rcc::gemm_tc_split(kind, M, N, Kpad, table != 0, scratch, sms, bn);
 }
