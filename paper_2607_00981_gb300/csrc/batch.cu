@@ -446,11 +446,8 @@ int run_once(rccsdt_batch* b) {
 
 #define RCC_API extern "C" __attribute__((visibility("default")))
 
-RCC_API int rccsdt_batch_create(int n, const int* o, const int* v, const int* naux, const rccsdt_options* opt,
-                                void* stream, rccsdt_batch** out) {
-  if (!out) return RCCSDT_ERR_ARG;
-  *out = nullptr;
-  if (n < 1 || !o || !v || !naux) return RCCSDT_ERR_ARG;
+static int batch_create(int n, const int* o, const int* v, const int* naux, const rccsdt_options* opt, void* stream,
+                        bool lean, rccsdt_batch** out) {
   rccsdt_options def;
   rccsdt_options_default(&def);
   auto* b = new rccsdt_batch();
@@ -462,7 +459,7 @@ RCC_API int rccsdt_batch_create(int n, const int* o, const int* v, const int* na
   int st = 0;
   for (int i = 0; i < n && !st; ++i) {
     rccsdt_ctx* c = nullptr;
-    st = rccsdt_create(o[i], v[i], naux[i], &b->opt, stream, &c);
+    st = rcc::ctx_create(o[i], v[i], naux[i], &b->opt, stream, lean, &c);
     if (!st) {
       b->inst.push_back(c);
       if (n > 1) st = rcc::ctx_set_concurrent(c, 1);
@@ -533,6 +530,16 @@ RCC_API int rccsdt_batch_create(int n, const int* o, const int* v, const int* na
   }
   *out = b;
   return RCCSDT_OK;
+}
+
+RCC_API int rccsdt_batch_create(int n, const int* o, const int* v, const int* naux, const rccsdt_options* opt,
+                                void* stream, rccsdt_batch** out) {
+  if (!out) return RCCSDT_ERR_ARG;
+  *out = nullptr;
+  if (n < 1 || !o || !v || !naux) return RCCSDT_ERR_ARG;
+  const int st = batch_create(n, o, v, naux, opt, stream, false, out);
+  // what the first instances hold to be faster must not keep the later ones out
+  return st == RCCSDT_ERR_OOM ? batch_create(n, o, v, naux, opt, stream, true, out) : st;
 }
 
 RCC_API rccsdt_ctx* rccsdt_batch_instance(rccsdt_batch* b, int i) {

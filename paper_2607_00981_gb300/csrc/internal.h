@@ -27,6 +27,8 @@ cudaStream_t ctx_stream(const rccsdt_ctx* c);
 void ctx_set_stream(rccsdt_ctx* c, cudaStream_t s);
 int ctx_main_precision(const rccsdt_ctx* c);
 void ctx_reset_precision(rccsdt_ctx* c);
+// rccsdt_create; lean: without what only makes a context faster (the waves' memory).
+int ctx_create(int o, int v, int naux, const rccsdt_options* opt, void* stream, bool lean, rccsdt_ctx** out);
 // 1: other contexts run concurrently on the GPU (a batch), so GEMMs are launched
 // with their natural grids instead of splitting K across every SM.  0, or an rccsdt_status.
 int ctx_set_concurrent(rccsdt_ctx* c, int on);

@@ -6,8 +6,11 @@
 // plain host loops over the same per-element functions (elem.cuh), so the host
 // logic can be checked against the oracle without a GPU.  The product binding
 // never loads it; the CUDA library has no CPU path.
+#include <malloc.h>
+
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <vector>
 
@@ -17,6 +20,20 @@
 namespace rcc {
 
 long long g_launch_count = 0;
+
+// The simulated device's memory: bytes in use, and a limit that a test may set (0: none).
+size_t g_live = 0, g_limit = 0;
+void* host_alloc(size_t bytes) {
+  if (g_limit && g_live + bytes > g_limit) return nullptr;
+  void* p = calloc(bytes ? bytes : 1, 1);
+  if (p) g_live += malloc_usable_size(p);
+  return p;
+}
+void host_free(void* p) {
+  if (p) g_live -= malloc_usable_size(p);
+  free(p);
+}
+
 // launches by form (test hook): gathering products, grouped FP64 products, grouped split products, grouped combines
 long long g_forms[4] = {0, 0, 0, 0};
 
@@ -91,7 +108,7 @@ int launch_gemm_tc(int kind, const void* Ahi, const void* Alo, const void* Bhi, 
         for (int k = k0; k < std::min(Kpad, k0 + len); ++k) {
           const i64 ia = (i64)m * Kpad + k, ib = (i64)n * Kpad + k;
           const float ah = get(Ahi, ia), al = get(Alo, ia), bh = get(Bhi, ib), bl = get(Blo, ib);
-          s += ah * bh + ah * bl + al * bh;
+          s += ah * bh + (ah * bl + al * bh);  // (the same for the transposed product)
         }
         sum += (double)s;
       }
@@ -399,7 +416,7 @@ int launch_gemm_tc_grouped(int kind, const GProblem* probs, int nprob, int, int,
           for (int k = z * len; k < std::min(P.Kpad, (z + 1) * len); ++k) {
             const i64 ia = (i64)m * P.Kpad + k, ib = (i64)n * P.Kpad + k;
             const float ah = get(P.a_hi, ia), al = get(P.a_lo, ia), bh = get(P.b_hi, ib), bl = get(P.b_lo, ib);
-            s += ah * bh + ah * bl + al * bh;
+            s += ah * bh + (ah * bl + al * bh);  // (the same for the transposed product)
           }
           P.out[P.colmajor ? (i64)n * P.M + m : ((i64)z * P.M + m) * P.N + n] = s;
         }
@@ -745,6 +762,12 @@ template void launch_t2_outer<float>(float*, const float*, const float*, const i
 extern "C" void rcc_test_f64_to_f32(const double* x, float* y, long long n) {
   for (long long i = 0; i < n; ++i) y[i] = rcc::f64_to_f32_rn(x[i]);
 }
+// Test hook: sets the limit (0: none); bytes in use.
+extern "C" long long rcc_test_memory(long long limit) {
+  rcc::g_limit = (size_t)limit;
+  return (long long)rcc::g_live;
+}
+
 // Test hook: launches by form since the last call.
 extern "C" void rcc_test_forms(long long* out) {
   for (int q = 0; q < 4; ++q) {
