@@ -1,5 +1,6 @@
 // Internal interface between the single-instance runtime and the batched driver.
 #pragma once
+#include "../../include/rccsdt.h"
 #include <cuda_runtime.h>
 
 #include <vector>
