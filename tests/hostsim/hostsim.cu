@@ -762,6 +762,21 @@ template void launch_t2_outer<float>(float*, const float*, const float*, const i
 extern "C" void rcc_test_f64_to_f32(const double* x, float* y, long long n) {
   for (long long i = 0; i < n; ++i) y[i] = rcc::f64_to_f32_rn(x[i]);
 }
+// Graph captures (bit 0) or launches (bit 1) that fail, for a test; replays since the last call.
+namespace rcc {
+int g_graph_fail = 0, g_replays = 0;
+bool host_graph_fails(int what) {
+  g_replays += what == 1 && !(g_graph_fail & 2);
+  return g_graph_fail >> what & 1;
+}
+}  // namespace rcc
+extern "C" int rcc_test_graphs(int fail) {
+  const int n = rcc::g_replays;
+  rcc::g_graph_fail = fail;
+  rcc::g_replays = 0;
+  return n;
+}
+
 // Test hook: sets the limit (0: none); bytes in use.
 extern "C" long long rcc_test_memory(long long limit) {
   rcc::g_limit = (size_t)limit;
