@@ -735,12 +735,6 @@ void launch_combine(const CombineArgs& c0, cudaStream_t s) {
 // 3 to 15 us; grouped by dependence they are about 20.  FP32 values are widened on the
 // integer path and plain copies skip the FP64 pipe.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double widen(float x) {  // exact, subnormals to zero
-  const unsigned u = __float_as_uint(x), e = u & 0x7f800000u;
-  const unsigned up = e == 0x7f800000u ? 0x70000000u : 0x38000000u;
-  const unsigned hi = e ? (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + up) : 0u;
-  return __longlong_as_double(((long long)hi << 32) | (long long)(e ? u << 29 : 0u));
-}
 
 // One step of kApplyTile outputs of a CTA.  IT is the type of element offsets, VEC: a
 // thread's four elements are consecutive (else 256 apart), loaded and stored together

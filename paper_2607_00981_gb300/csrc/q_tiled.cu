@@ -20,14 +20,15 @@
 // as fma.f32x2.  A tile is stored to a shared buffer of its own (no two writers per
 // element) and every thread then adds, in a fixed order, the permuted elements of its
 // occupied tuples into registers.  The spin sum t~ has coefficients +-2^n and is unrolled
-// with the permuted offsets as sums of compile-time multiples; FP32 takes it, and the
-// division by the energy denominators, in double-float (FP64 for those, 24 conversions
-// and multiply-adds and a division per tuple, cost more than all products).
+// with the permuted offsets as sums of compile-time multiples; FP32 takes it as a
+// sum of three floats (error-free additions, about 70 bits; 24 FP64 additions per tuple made
+// o=6 v=48 74.6 ms); the quotients by the energy denominators and every sum of energies
+// are FP64.  (In two floats, with the quotients, 62.9 ms; now 69.1.)
 //
 // FP64 is bound by its pipe (41 ms at o=5 v=29 against 84 ms for 24 permutations).  FP32
 // is bound by shared memory (16-byte row loads feeding two columns each) and by the
-// latency between its barriers at two CTAs per SM: o=6 v=48, 247596 quadruples, 57 ms
-// (14.6 TFLOP/s executed) against 589 ms for the permutation-by-permutation kernel; the
+// latency between its barriers at two CTAs per SM: o=6 v=48, 247596 quadruples, 63 ms
+// (13.2 TFLOP/s executed) against 589 ms for the permutation-by-permutation kernel; the
 // intermediates with it 5.4 ms against 32 ms.
 #include <cuda_runtime.h>
 
@@ -35,6 +36,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "elem.cuh"
 #include "q_tiled.h"
 
 namespace rcc {
@@ -387,10 +389,10 @@ __device__ __forceinline__ void copy_wait(int pending) {  // at most `pending` g
   else asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-__device__ __forceinline__ void two_sum(float& h, float& l, float x) {  // (h, l) += x
-  const float s = h + x, bp = s - h;
-  l += (h - (s - bp)) + (x - bp);
+__device__ __forceinline__ float two_sum(float& h, float x) {  // h += x; what its rounding leaves
+  const float s = h + x, bp = s - h, e = (h - (s - bp)) + (x - bp);
   h = s;
+  return e;
 }
 
 template <typename T, int O>
@@ -401,8 +403,8 @@ __global__ void __launch_bounds__(qt_threads(O), qt_min_ctas<T>(O)) k_qt_main(co
   extern __shared__ __align__(16) unsigned char qt_smem[];
   const int v = a.v, tid = threadIdx.x;
   T* buf = (T*)qt_smem;
-  T* seps = buf + C::BUF;           // sum of the occupied energies of a tuple (FP32: hi, lo)
-  T* xs = seps + C::EPS;            // sums over the rounds, each tuple's by its own thread
+  double* seps = (double*)(buf + C::BUF);  // sum of the occupied energies of a tuple
+  T* xs = buf + C::BUF + C::EPS;    // sums over the rounds, each tuple's by its own thread
   T* ys = xs + C::O4P;
   T* Vs = ys + C::O4P;              // [6][O2] integrals, [6][O2] t2
   T* A2s = Vs + C::VST;             // [4][i][m][OP]
@@ -476,12 +478,7 @@ __global__ void __launch_bounds__(qt_threads(O), qt_min_ctas<T>(O)) k_qt_main(co
   };
   for (int el = tid; el < O4; el += TH) {
     const double e = a.eps[el / O3] + a.eps[el / O2 % O] + a.eps[el / O % O] + a.eps[el % O];
-    if constexpr (sizeof(T) == 4) {
-      seps[2 * el] = (float)e;
-      seps[2 * el + 1] = (float)(e - (double)(float)e);
-    } else {
-      seps[el] = e;
-    }
+    seps[el] = e;
   }
   if (tid == 0) next(blockIdx.x, 0);
   __syncthreads();
@@ -747,9 +744,7 @@ __global__ void __launch_bounds__(qt_threads(O), qt_min_ctas<T>(O)) k_qt_main(co
     if (sqi[par ^ 1] < a.ntuple) prefetch(par ^ 1);  // flies over the spin sum
     __syncthreads();
     const double ev = a.eps[O + L[0]] + a.eps[O + L[1]] + a.eps[O + L[2]] + a.eps[O + L[3]];
-    const float evh = (float)ev, evl = (float)(ev - (double)evh);
     double part = 0.0;
-    float fhi = 0.f, flo = 0.f;
 #pragma unroll 1
     for (int el = tid; el < O4; el += TH) {
       const int oc[4] = {el / O3, el / O2 % O, el / O % O, el % O};
@@ -765,25 +760,18 @@ __global__ void __launch_bounds__(qt_threads(O), qt_min_ctas<T>(O)) k_qt_main(co
 #pragma unroll
       for (int q = 0; q < 4; ++q) mu[q][0] = oc[q], mu[q][1] = oc[q] * O, mu[q][2] = oc[q] * O2, mu[q][3] = oc[q] * O3;
       auto at = [&](int i0, int i1, int i2, int i3) { return buf[mu[i0][3] + mu[i1][2] + mu[i2][1] + mu[i3][0]]; };
+      double s = 0.0;
       if constexpr (sizeof(T) == 8) {
-        double s = 0.0;
         each_ordering([&](int c, int i0, int i1, int i2, int i3) { s = fma((double)c, at(i0, i1, i2, i3), s); });
         part += z * s / (seps[el] - ev);
-      } else {
-        float hi = 0.f, lo = 0.f;
-        each_ordering([&](int c, int i0, int i1, int i2, int i3) { two_sum(hi, lo, (float)c * at(i0, i1, i2, i3)); });
-        // (z t~) / eps in double-float: eps and its reciprocal as float pairs
-        float dh = seps[2 * el], dl = seps[2 * el + 1];
-        two_sum(dh, dl, -evh);
-        dl -= evl;
-        const float q = 1.0f / dh, ql = q * (fmaf(-q, dh, 1.0f) - q * dl);
-        const float ph = hi * z, pl = fmaf(hi, z, -ph) + lo * z;
-        const float mh = ph * q, ml = fmaf(ph, q, -mh) + (pl * q + ph * ql);
-        two_sum(fhi, flo, mh);
-        flo += ml;
+      } else {  // (the coefficients are powers of two)
+        float h = 0.f, m = 0.f, l = 0.f;
+        each_ordering([&](int c, int i0, int i1, int i2, int i3) {
+          l += two_sum(m, two_sum(h, (float)c * at(i0, i1, i2, i3)));
+        });
+        part += widen(z) * (widen(h) + (widen(m) + widen(l))) / (seps[el] - ev);
       }
     }
-    if constexpr (sizeof(T) == 4) part = (double)fhi + (double)flo;
     total += (double)fac * part;
   }
 #pragma unroll
