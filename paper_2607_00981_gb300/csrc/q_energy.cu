@@ -803,15 +803,15 @@ int q_energy(rccsdt_ctx* ctx, const rcc::QInputs& in, double* e_q, double* info)
   const int smem = in_smem ? (int)rz_bytes : 0;
   ++rcc::g_launch_count;
   if (staged) {
-    auto launch = [&](auto kern) {
-      if (staged_bytes > 48 * 1024)
+    if constexpr (sizeof(T) == 4) {  // o = 1 and o >= 9: the others take the tiled form
+      auto launch = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged_bytes);
-      kern<<<grid, kThreadsQ, staged_bytes, s>>>(qa);
-    };
-    if (o <= 4) launch(k_q_main_staged<T, 4>);
-    else if (o <= 8) launch(k_q_main_staged<T, 8>);
-    else if (o <= 12) launch(k_q_main_staged<T, 12>);
-    else launch(k_q_main_staged<T, 16>);
+        kern<<<grid, kThreadsQ, staged_bytes, s>>>(qa);
+      };
+      if (o <= 4) launch(k_q_main_staged<T, 4>);
+      else if (o <= 12) launch(k_q_main_staged<T, 12>);
+      else launch(k_q_main_staged<T, 16>);
+    }
   } else {
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_q_main<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     k_q_main<T><<<grid, kThreadsQ, smem, s>>>(qa);

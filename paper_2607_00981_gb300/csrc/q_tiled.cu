@@ -1,4 +1,5 @@
-// RCCSDT(Q) for 2 <= o <= 8: the ABC-ordered sum of q_energy.cu (same equations and
+// RCCSDT(Q) for small o (2 <= o <= 8 in FP32; in FP64, whose tiles are twice the size in shared
+// memory, 2 <= o <= 6, and o = 7 up to v = 86): the ABC-ordered sum of q_energy.cu (same equations and
 // notation) with the products of one virtual quadruple as register-tiled GEMMs.
 //
 // Each of the four products of r = P(X + Y) is symmetric under one exchange of its
@@ -297,11 +298,17 @@ struct QtArgs {
   double* partial;  // [grid]
 };
 
-// threads per CTA (about the items of one X round) and CTAs per SM the registers allow
+// Threads per CTA: the items of one X round, 2 ceil(o^3 / 2), in whole warps; half of them for
+// o = 8 (512), where 512 threads would leave 128 registers, less than the tiles take.  CTAs
+// per SM that the registers are cut for: as many as their threads fill (FP32, o <= 4), then
+// as many as shared memory takes (o = 5 four, o = 6 two, o >= 7 one; FP64 one from o = 5 on).
+// Against a thread per tuple with 24 permutations: o = 2, v = 60 16.4 ms (463), o = 3, v = 20
+// 0.54 (4.4), o = 4, v = 30 2.6 (27.1), o = 5, v = 30 6.1 (42.4), o = 7, v = 24 9.2 (43.4), o = 8,
+// v = 20 6.5 (41.1); in FP64 o = 6, v = 20 16.4 (36.8).
 constexpr int qt_threads(int O) { return O <= 3 ? 32 : O == 4 ? 64 : O == 5 ? 128 : O == 6 ? 224 : O == 7 ? 352 : 256; }
 template <typename T>
 constexpr int qt_min_ctas(int O) {
-  return sizeof(T) == 8 ? (O <= 4 ? 4 : 1) : O <= 3 ? 16 : O == 4 ? 8 : O == 5 ? 4 : O == 7 ? 1 : 2;
+  return sizeof(T) == 8 ? (O <= 4 ? 4 : 1) : O <= 3 ? 16 : O == 4 ? 8 : O == 5 ? 4 : O == 6 ? 2 : 1;
 }
 constexpr int kQtEC = 16;  // e values staged at a time in phase Y
 
@@ -830,9 +837,10 @@ size_t smem_of(int o, int v) {
     case 5: return QtCfg<T, 5>::smem(v, 1);
     case 6: return QtCfg<T, 6>::smem(v, 1);
     case 7: return QtCfg<T, 7>::smem(v, 1);
-    case 8: return QtCfg<T, 8>::smem(v, 1);
+    case 8:
+      if constexpr (sizeof(T) == 4) return QtCfg<T, 8>::smem(v, 1);  // (FP64: 320 KB)
   }
-  return ~(size_t)0;
+  return (size_t)1 << 40;  // does not fit
 }
 
 }  // namespace
@@ -931,7 +939,9 @@ int qt_main(const QtInputs& in, char* ws, const QtSizes& z, int nsm, int smem_ma
     case 5: st = launch_main<T, 5>(a, nsm, smem_max, grid, s); break;
     case 6: st = launch_main<T, 6>(a, nsm, smem_max, grid, s); break;
     case 7: st = launch_main<T, 7>(a, nsm, smem_max, grid, s); break;
-    case 8: st = launch_main<T, 8>(a, nsm, smem_max, grid, s); break;
+    case 8:
+      if constexpr (sizeof(T) == 4) st = launch_main<T, 8>(a, nsm, smem_max, grid, s);
+      break;
   }
   if (st) return 1;
   ++g_launch_count;
