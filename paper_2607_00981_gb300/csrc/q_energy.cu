@@ -813,7 +813,8 @@ int q_energy(rccsdt_ctx* ctx, const rcc::QInputs& in, double* e_q, double* info)
       else launch(k_q_main_staged<T, 16>);
     }
   } else {
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_q_main<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // (the static tables count against the 48 KB that need no opt-in)
+    if (smem) cudaFuncSetAttribute(k_q_main<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     k_q_main<T><<<grid, kThreadsQ, smem, s>>>(qa);
   }
   cudaEventRecord(ev[3], s);
