@@ -95,3 +95,21 @@ def test_waves_are_bitwise_the_products_one_by_one(prec, o, v, naux):
         ctx.close()
     for x, y in zip(*out):
         assert np.array_equal(x, y)
+
+
+def test_digit_planes_do_not_grow_with_the_panels():
+    """The planes are cut from the plans' own operands, not from what the waves add."""
+    lib = hostsim_lib()
+    o, v, naux = 2, 12, 168
+    base, held = _memory(lib, 0), {}
+    for f64_tc in (0, 1):
+        for lean in (False, True):
+            _memory(lib, base + used - 300000 if lean else 0)
+            try:
+                ctx = B.Context(lib, o, v, naux, precision=B.SPLIT_BF16X3, diis_space=2, f64_tc=f64_tc)
+            finally:
+                used = _memory(lib, 0) - base
+            held[f64_tc, lean] = ctx.device_bytes()
+            ctx.close()
+    assert held[0, True] < held[0, False]
+    assert held[1, False] - held[0, False] == held[1, True] - held[0, True] > 0
