@@ -6,8 +6,8 @@
 
 namespace rcc {
 
-constexpr int kDotBlocks = 608;
-extern long long g_launch_count;  // 4 x 152 SMs, fixed so reductions are deterministic
+constexpr int kDotBlocks = 608;  // 4 x 152 SMs, fixed so reductions are deterministic
+extern long long g_launch_count;
 
 struct CombineArgs {
   double* out;
