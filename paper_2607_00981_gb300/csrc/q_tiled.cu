@@ -816,8 +816,8 @@ int launch_main(QtArgs<T> a, int nsm, int smem_max, int* grid, cudaStream_t s) {
   const size_t smem = QtCfg<T, O>::smem(a.v, a.nx);
   if (smem + 2048 > (size_t)smem_max) return 1;
   int per_sm = 0;
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(k_qt_main<T, O>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  // (always: the static tables count against the 48 KB that need no opt-in)
+  if (cudaFuncSetAttribute(k_qt_main<T, O>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return 1;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_qt_main<T, O>, qt_threads(O), smem) != cudaSuccess ||
       per_sm < 1)
